@@ -171,7 +171,7 @@ __device__ __forceinline__ float* entry_layers(float* tile, float* tmp, const fl
             s += tile[e + dy * R + dx];
       if constexpr (BIAS) s += b;
       const float2 p = pt[i * R + k], q = qt[i2 * R + k2];
-      const float c = s * (p.x * q.x);
+      const float c = __saturatef(s * (p.x * q.x));
       tmp[e] = (p.y * q.y) * f2_lo(nk_Jpi01_2(f2_make(c, c)));
     }
     sync();

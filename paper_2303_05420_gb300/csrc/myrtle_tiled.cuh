@@ -468,12 +468,13 @@ struct Band {
       if constexpr (BIAS) K = f2_add(K, f2_dup(b));
       const float2 p = pv[k], q0 = qh[j][k], q1 = lds64(qa[k] + qo);
       qh[j][k] = q1;
-      const f2 c = f2_mul(K, f2_make(p.x * q0.x, p.x * q1.x));
+      constexpr bool SIGNED = ACT == NK_ACT_ERF || (SEED && j == 0);  // correlations may be negative
+      const f2 aa = f2_make(p.x * q0.x, p.x * q1.x), c = SIGNED ? f2_mul(K, aa) : f2_mul_sat(K, aa);
       f2 J;
       if constexpr (ACT == NK_ACT_ERF)
         J = nk_asin_2(c);  // Erf: (2/pi) asin(c), 2/pi folded into the p side
       else
-        J = (SEED && j == 0) ? nk_Jpi_2(c) : nk_Jpi01_2(c);
+        J = SIGNED ? nk_Jpi_2(c) : nk_Jpi01_2(c);
       const f2 sq = f2_make(p.y * q0.y, p.y * q1.y);
       A[k] = f2_mul(sq, J);
       if constexpr (NTK) {

@@ -41,6 +41,11 @@ __device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(a.u), "l"(b.u));
   return r;
 }
+// a b clamped to [0, 1] (0 for a NaN): the clamp is the scalar
+// multiplication's own, which the packed one has not.
+__device__ __forceinline__ f2 f2_mul_sat(f2 a, f2 b) {
+  return f2_make(__saturatef(f2_lo(a) * f2_lo(b)), __saturatef(f2_hi(a) * f2_hi(b)));
+}
 __device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
   f2 r;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(a.u), "l"(b.u));
@@ -78,24 +83,27 @@ __device__ __forceinline__ f2 nk_Bpi_poly2(f2 c) {
   return p;
 }
 
-// u sqrt|u| on both halves.  u = 1 - c is below zero only where c exceeds 1
-// by rounding; there |u|^{3/2} is under the rounding of J, so the magnitude
-// (a free operand modifier) replaces the clamp c <= 1 of the scalar form.
+// u sqrt(u) on both halves, u >= 0.
 __device__ __forceinline__ f2 nk_u32(f2 u) {
-  return f2_mul(u, f2_make(nk_sqrt_approx(fabsf(f2_lo(u))), nk_sqrt_approx(fabsf(f2_hi(u)))));
+  return f2_mul(u, f2_make(nk_sqrt_approx(f2_lo(u)), nk_sqrt_approx(f2_hi(u))));
 }
 
-// J(c) / pi for c >= 0 on both halves (nk_J01_f32).
+// J(c) / pi for c in [0, 1] on both halves (nk_J01_f32).  The caller clamps
+// (f2_mul_sat): c = K a a' is above 1 not only by rounding, and the polynomial
+// has no bound there.  Where sqrt(q q') < 2.9e-39 the product a a' of the
+// factors 1 / sqrt(q) is infinite, c infinite or (K = 0) a NaN, and such a
+// pixel pair, which adds b b' J ~ 1e-39, would spoil the whole entry.
 __device__ __forceinline__ f2 nk_Jpi01_2(f2 c) {
   return f2_fma(nk_u32(f2_sub(KONE, c)), nk_Bpi_poly2(c), c);
 }
 
-// J(c) / pi for any c on both halves (nk_J_f32): J(|c|) + pi min(c, 0) =
-// pi max(c, 0) + (1 - |c|)^{3/2} B(|c|).
+// J(c) / pi for any c on both halves (nk_J_f32; c beyond [-1, 1] counts as the
+// nearer end, a NaN gives 0): J(|c|) + pi min(c, 0) = pi max(c, 0) + (1 -
+// |c|)^{3/2} B(|c|).
 __device__ __forceinline__ f2 nk_Jpi_2(f2 c) {
   const float c0 = f2_lo(c), c1 = f2_hi(c);
-  const f2 a = f2_make(fabsf(c0), fabsf(c1));
-  return f2_fma(nk_u32(f2_sub(KONE, a)), nk_Bpi_poly2(a), f2_make(fmaxf(c0, 0.f), fmaxf(c1, 0.f)));
+  const f2 a = f2_make(fminf(fabsf(c0), 1.f), fminf(fabsf(c1), 1.f));
+  return f2_fma(nk_u32(f2_sub(KONE, a)), nk_Bpi_poly2(a), f2_make(__saturatef(c0), __saturatef(c1)));
 }
 
 // asin(c) for c in [-1, 1] (nk_asin_f32; values outside by rounding act as
