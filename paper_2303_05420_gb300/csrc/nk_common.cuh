@@ -76,6 +76,23 @@ nk_status nk_cuda_check(nk_handle* h, cudaError_t e, const char* what);
 nk_status nk_workspace(nk_handle* h, size_t bytes, void** out);
 void nk_pcg_free_host(nk_handle* h);
 
+// Opts a kernel in to `dynamic` bytes of shared memory a block.  Without it
+// dynamic and static bytes together must fit 48 KB, so a kernel with static
+// tables needs it from fewer dynamic bytes on: asked for from 32 KB, which
+// leaves 16 for them.  The limit is set to all that the kernel's static bytes
+// leave (227 KB), never back: another host thread may be between its own
+// request and its launch.
+template <class K>
+inline cudaError_t nk_smem_optin(K kernel, size_t dynamic) {
+  if (dynamic <= 32 * 1024) return cudaSuccess;
+  cudaFuncAttributes a;
+  cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+  if (e != cudaSuccess) return e;
+  const int most = 227 * 1024 - (int)a.sharedSizeBytes;
+  if (a.maxDynamicSharedSizeBytes >= most) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // Launchers (each returns a CUDA error, arguments already validated).
 size_t nk_self_diag_ws_bytes(const NkGeom& g, int64_t n);
 cudaError_t nk_launch_self_diag(const NkGeom& g, double sw2, double sb2, const float* X, int64_t n, double* qd,

@@ -272,8 +272,7 @@ cudaError_t nk_launch_self_adj(const NkGeom& g, double sw2, double sb2, const fl
         const int halo = g.filter / 2 * g.convs[s] + g.radius[s];
         const int bands = nk_self_bands(H, W, m * (G.nh[s] - 1), halo, 3, sm);
         const size_t psm = 3 * (size_t)std::min(H, (H + bands - 1) / bands + 2 * halo) * W * sizeof(double);
-        if (psm > 48 * 1024)
-          e = cudaFuncSetAttribute(k_self_adj_planes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm);
+        e = nk_smem_optin(k_self_adj_planes, psm);
         if (e != cudaSuccess) return e;
         ++*launches;
         k_self_adj_planes<<<dim3((unsigned)bands, (unsigned)(G.nh[s] - 1), (unsigned)m), 256, psm, st>>>(
@@ -281,8 +280,7 @@ cudaError_t nk_launch_self_adj(const NkGeom& g, double sw2, double sb2, const fl
       }
       const int chalo = g.filter / 2 * g.convs[s], cb = nk_self_bands(H, W, m, chalo, 2, sm);
       const size_t csm = 2 * (size_t)(cb == 1 ? H : std::min(H, (H + cb - 1) / cb + 2 * chalo)) * W * sizeof(double);
-      if (csm > 48 * 1024)
-        e = cudaFuncSetAttribute(k_self_adj_center<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm);
+      e = nk_smem_optin(k_self_adj_center<T>, csm);
       if (e != cudaSuccess) return e;
       ++*launches;
       k_self_adj_center<T><<<dim3((unsigned)m, (unsigned)cb), 512, csm, st>>>(G, s, cb, sw2, sb2, B, A,

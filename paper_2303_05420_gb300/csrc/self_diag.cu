@@ -226,8 +226,7 @@ cudaError_t nk_self_forward(const SelfGeom& G, double sw2, double sb2, const flo
     const int crows = cb == 1 ? g.Hs[s] : std::min(g.Hs[s], (g.Hs[s] + cb - 1) / cb + 2 * halo);
     const size_t csm = (2 * (size_t)crows * g.Ws[s] + 33) * sizeof(double);
     auto kc = store ? k_self_center<true> : k_self_center<false>;
-    cudaError_t e = cudaSuccess;
-    if (csm > 48 * 1024) e = cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm);
+    cudaError_t e = nk_smem_optin(kc, csm);
     if (e != cudaSuccess) return e;
     ++*launches;
     kc<<<dim3((unsigned)m, (unsigned)cb), 512, csm, st>>>(G, s, cb, sw2, sb2, X, B, qd, qs, dstatus);
@@ -236,7 +235,7 @@ cudaError_t nk_self_forward(const SelfGeom& G, double sw2, double sb2, const flo
       const int rows = std::min(g.Hs[s], (g.Hs[s] + bands - 1) / bands + 2 * halo);
       const size_t psm = 2 * (size_t)rows * g.Ws[s] * sizeof(double);
       auto kp = store ? k_self_planes<true> : k_self_planes<false>;
-      if (psm > 48 * 1024) e = cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm);
+      e = nk_smem_optin(kp, psm);
       if (e != cudaSuccess) return e;
       ++*launches;
       kp<<<dim3((unsigned)bands, (unsigned)(G.nh[s] - 1), (unsigned)m), 256, psm, st>>>(G, s, bands, sw2, sb2, X, B);
