@@ -9,16 +9,25 @@
 // sums went through it twice.  Here K is read once per run, a row's product
 // sums stay on its SM, and what an iteration costs is crossing the chip.
 //
-// So it is CG with one reduction (Chronopoulos and Gear, 1989): with u = M r
-// and w = A u the sums (r, u), (r, r) and (w, u) are taken together, s = A p
-// follows p's own recurrence and (p, A p) is (w, u) - beta^2 (p, A p)_old.  An
-// iteration crosses the chip twice, about 3 us each: u is published, the sums
-// are collected; the textbook form's third crossing (the direction, after
-// beta) is gone: 15.4 -> 12.7 us an iteration at N = 2048, 10 columns.  Flags
-// in place of the barriers (a warp waiting for the CTAs that own its columns,
-// a column for its own counter) were slower, 18: every word has 152 pollers.
+// Textbook CG needs three crossings an iteration, about 3 us each: the sum that
+// beta takes, the direction, (p, A p).  Where a warp has one block of columns
+// and one group of right-hand sides (KEEP: N up to about 2,700 and 16 columns,
+// 10 from N = 2,049 on) two do: z = M r is published together with (r, z) and
+// (r, r), and after that crossing every SM forms the direction p = z + beta
+// p_old on its own, its old one still in the lanes' registers.  It is the same
+// FP32 operation on the same values everywhere, so the p that the rows' owners
+// add to x is the p of the product.  Elsewhere the owners publish p.
 //
-// Matvec: a warp owns 128 columns; a lane holds u at 8 of them for half of a
+// CG with one reduction (Chronopoulos and Gear: A p and (p, A p) by recurrences)
+// has two crossings everywhere and was faster (12.7 us an iteration at N = 2048,
+// 10 columns, and 13.5 here), but with FP32 products its recurrences drift: at
+// kappa = 7e7 (1000 points, Gaussian kernel) (p, A p) came out negative and
+// the solve diverged where this form converges as the graph-replayed run does.
+// Flags in place of the barriers (a warp waiting for the CTAs that own its
+// columns, a column for its own counter) were slower, 18 us: every word has 152
+// pollers.
+//
+// Matvec: a warp owns 128 columns; a lane holds p at 8 of them for half of a
 // group of right-hand sides (2 RH <= 16 of them) in registers, as f32x2 over
 // column pairs, and meets every row of the CTA with two 16-byte loads.  A
 // row's sums over a warp's 128 columns are eight-column sums added in an FP32
@@ -49,15 +58,15 @@ struct Args {
   const double* B;
   const double* minv;
   double* X;
-  float* P;             // published u, see p_index
-  double* sums;         // [3 slots][R][4]: (r, u), (r, r), (w, u), unused
+  float* P;             // published z (KEEP) or p, see p_index
+  double* sums;         // [3 slots][R][4]: (r, z), (r, r), (p, A p), unused
   unsigned* bar;        // barrier count; bar[1]: status
   double lam, tol2;
   int maxit;
   double* iters;        // [R] iterations of each column
 };
 
-// Element (i, r) of the published u: right-hand sides in groups of
+// Element (i, r) of the published vector: right-hand sides in groups of
 // 2 RH, within a group blocks of 8 columns x RH sides per (8-column block,
 // half), which is what a lane loads.
 template <int RH>
@@ -109,7 +118,9 @@ __device__ __forceinline__ void two_sum(float& s, float& c, float p) {
 }
 
 // STREAM: rows from a.res on are read from memory in every product.
-template <int RH, int MAXT, bool STREAM>
+// KEEP: a warp has one block of columns and one group of right-hand sides, and
+// its lanes keep their p in registers.
+template <int RH, int MAXT, bool STREAM, bool KEEP>
 __global__ void __launch_bounds__(MAXT, 1) k_cg_resident(const __grid_constant__ Args a) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int RC = 16 / RH, V = RC * RH;  // rows a butterfly folds; its values (<= 16)
@@ -122,20 +133,18 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_resident(const __grid_constant__
   double* x = reinterpret_cast<double*>(Ks + (size_t)a.res * npad);
   double* rv = x + a.nr * R;
   double* p = rv + a.nr * R;
-  double* s = p + a.nr * R;
-  double* u = s + a.nr * R;
-  double* wv = u + a.nr * R;
-  double* mi = wv + a.nr * R;                       // [nr]
-  float* part = reinterpret_cast<float*>(mi + a.nr + (a.nr & 1));  // [cbs][nr * 2 RH]
+  double* q = p + a.nr * R;
+  double* mi = q + a.nr * R;                              // [nr]
+  float* pf = reinterpret_cast<float*>(mi + a.nr);        // [R][nr]: p again, and z
+  float* zf = pf + a.nr * R;
+  float* part = zf + a.nr * R;                            // [cbs][nr * 2 RH]
   const int pstride = a.nr * 2 * RH;
   // this thread's row and its first column; the columns repeat every cstep
   const int ri = lane & (a.gl - 1), col0 = warp * (32 / a.gl) + lane / a.gl, cstep = (T >> 5) * (32 / a.gl);
-  // column `lane` in warp 0: (r, u), its reciprocal and (p, A p) of the last
-  // iteration, tol^2 (b, b), iterations, whether it goes on
-  double c_ru = 0.0, c_inv = 0.0, c_pq = 0.0, c_lim = 0.0;
-  int c_its = 0;
-  bool c_on = tid < R;
-  __shared__ double s_al[32], s_be[32];
+  int c_its = 0;  // iterations of column `lane`, warp 0
+  // per column: alpha, beta, 1 / (r, z), tol^2 (b, b), whether it goes on
+  __shared__ double s_al[32], s_inv[32], s_lim[32];
+  __shared__ float s_be[32];
   __shared__ int s_on[32];
   GridBarrier gb = {a.bar, 0, true};
 
@@ -156,6 +165,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_resident(const __grid_constant__
     }
   }
   for (int i = tid; i < nrow; i += T) mi[i] = a.minv[row0 + i];
+  if (tid < 32) {
+    s_inv[tid] = s_lim[tid] = 0.0;
+    s_on[tid] = tid < R;
+  }
   __syncthreads();
 
   // sum over a column's lanes (every lane of the warp takes part)
@@ -163,15 +176,15 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_resident(const __grid_constant__
     for (int o = a.gl >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
   };
-  // u = M r is published, (r, u) and (r, r) go to slot `slot`
+  // z = M r (published with KEEP); (r, z) and (r, r) go to slot `slot`
   auto publish = [&](int r, bool mine, int slot) {
-    double ru = 0.0, rr = 0.0;
+    double rz = 0.0, rr = 0.0;
     if (mine) {
       const int e = r * a.nr + ri;
-      const double rn = rv[e], un = mi[ri] * rn;
-      u[e] = un;
-      __stcg(a.P + p_index<RH>(npad, row0 + ri, r), (float)un);
-      ru = rn * un;
+      const double rn = rv[e], zn = mi[ri] * rn;
+      zf[e] = (float)zn;
+      if constexpr (KEEP) __stcg(a.P + p_index<RH>(npad, row0 + ri, r), zf[e]);
+      rz = rn * zn;
       rr = rn * rn;
     }
     // both sums in one butterfly: the upper half of the lanes takes (r, r)
@@ -179,13 +192,13 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_resident(const __grid_constant__
     double* out = a.sums + ((size_t)slot * R + min(r, R - 1)) * 4;
     if (o == 0) {
       if (mine) {
-        red_add(out, ru);
+        red_add(out, rz);
         red_add(out + 1, rr);
       }
       return;
     }
     const bool up = (ri & o) != 0;
-    double v = (up ? rr : ru) + __shfl_xor_sync(0xffffffffu, up ? ru : rr, o);
+    double v = (up ? rr : rz) + __shfl_xor_sync(0xffffffffu, up ? rz : rr, o);
     for (int x = o >> 1; x > 0; x >>= 1) v += __shfl_xor_sync(0xffffffffu, v, x);
     if (r < R && (ri & (o - 1)) == 0) red_add(out + (up ? 1 : 0), v);
   };
@@ -195,34 +208,82 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_resident(const __grid_constant__
     if (mine) {
       const int e = r * a.nr + ri;
       x[e] = 0.0;
-      p[e] = 0.0;
-      s[e] = 0.0;
+      pf[e] = 0.f;
       rv[e] = a.B[(int64_t)(row0 + ri) * R + r];
     }
     publish(r, mine, 0);
   }
 
+  // a lane's columns and right-hand sides of the published vector, block cb, group g
+  const int cg = lane >> 1, half = lane & 1;
+  auto at = [&](int g, int cb) {
+    return (int64_t)g * npad * 2 * RH + ((int64_t)((cb * 16 + cg) * 2 + half) * RH) * 8;
+  };
+  auto load = [&](const float* from, int h, f2 (&v)[4]) {
+    const float4 a = __ldcg(reinterpret_cast<const float4*>(from) + 2 * h);
+    const float4 b = __ldcg(reinterpret_cast<const float4*>(from) + 2 * h + 1);
+    v[0] = f2_make(a.x, a.y);
+    v[1] = f2_make(a.z, a.w);
+    v[2] = f2_make(b.x, b.y);
+    v[3] = f2_make(b.z, b.w);
+  };
+  f2 P2[RH][4];
+#pragma unroll
+  for (int h = 0; h < RH; ++h) P2[h][0] = P2[h][1] = P2[h][2] = P2[h][3] = f2_dup(0.f);
+
   for (int it = 0;; ++it) {
-    const int running = gb.arrive(c_on);
-    // off the path to the next sums: the reciprocal that beta takes
-    if (warp == 0 && it > 0) c_inv = fabs(c_ru) > 1e-300 ? 1.0 / c_ru : 0.0;
+    gb.arrive(0);
     if (!gb.leave()) return;
-    if (!running || it == a.maxit) break;
-    // w = (K + lam I) u, and (w, u)
+    // with registers to spare, z is on its way while the sums are
+    constexpr bool EARLY = KEEP && RH <= 5 && MAXT <= 512;
+    f2 Z2[EARLY ? RH : 1][4];
+    if constexpr (EARLY) {
+      if (warp < cbs) {
+#pragma unroll
+        for (int h = 0; h < RH; ++h) load(a.P + at(0, warp), h, Z2[h]);
+      }
+    }
     double* sums = a.sums + (size_t)(it % 3) * R * 4;
+    // every warp: the columns that go on (the same everywhere), and their beta;
+    // sums of squares compare as their bits do (a NaN stops its column)
+    double rz = 0.0;
+    int on = 0;
+    if (lane < R) {
+      const long long rr = __double_as_longlong(__ldcg(sums + lane * 4 + 1));
+      rz = __ldcg(sums + lane * 4);
+      on = s_on[lane] && (it == 0 || (rr > __double_as_longlong(s_lim[lane]) && rr <= 0x7ff0000000000000ll));
+    }
+    if (!__any_sync(0xffffffffu, on) || it == a.maxit) break;
+    const float beta = lane < R ? (float)(rz * s_inv[lane]) : 0.f;
+    if (warp == 0) s_be[lane] = beta;
+    if constexpr (!KEEP) {
+      __syncthreads();
+      for (int r = col0; r < R; r += cstep) {
+        const int e = r * a.nr + ri;
+        if (ri < nrow) __stcg(a.P + p_index<RH>(npad, row0 + ri, r), pf[e] = fmaf(s_be[r], pf[e], zf[e]));
+      }
+      gb.arrive(0);
+      if (!gb.leave()) return;
+    }
+    // A p and (p, A p), A = K + lam I
     for (int g = 0; g < a.groups; ++g) {
       for (int cb = warp; cb < cbs; cb += T >> 5) {
-        const int cg = lane >> 1, half = lane & 1;
-        f2 P2[RH][4];
-        const float4* src = reinterpret_cast<const float4*>(
-            a.P + (int64_t)g * npad * 2 * RH + ((int64_t)((cb * 16 + cg) * 2 + half) * RH) * 8);
 #pragma unroll
         for (int h = 0; h < RH; ++h) {
-          const float4 b0 = __ldcg(src + 2 * h), b1 = __ldcg(src + 2 * h + 1);
-          P2[h][0] = f2_make(b0.x, b0.y);
-          P2[h][1] = f2_make(b0.z, b0.w);
-          P2[h][2] = f2_make(b1.x, b1.y);
-          P2[h][3] = f2_make(b1.z, b1.w);
+          if constexpr (KEEP) {
+            f2 z[4];
+            if constexpr (EARLY) {
+#pragma unroll
+              for (int c = 0; c < 4; ++c) z[c] = Z2[h][c];
+            } else {
+              load(a.P + at(g, cb), h, z);
+            }
+            const f2 be = f2_dup(__shfl_sync(0xffffffffu, beta, half * RH + h));
+#pragma unroll
+            for (int c = 0; c < 4; ++c) P2[h][c] = f2_fma(be, P2[h][c], z[c]);
+          } else {
+            load(a.P + at(g, cb), h, P2[h]);
+          }
         }
         const int c0 = cb * 128 + cg * 8;
         float* out = part + (size_t)cb * pstride;
@@ -300,53 +361,49 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_resident(const __grid_constant__
       const int r0 = g * 2 * RH;
       for (int cw = warp * (32 / a.gl), r = col0; cw < R; cw += cstep, r += cstep) {
         const bool mine = r >= r0 && r < min(R, r0 + 2 * RH) && ri < nrow;
-        double wu = 0.0;
+        double pq = 0.0;
         if (mine) {
           float t = 0.f, c = 0.f;
           for (int w = 0; w < cbs; ++w) two_sum(t, c, part[(size_t)w * pstride + ri * 2 * RH + r - r0]);
           const int e = r * a.nr + ri;
-          const double un = u[e], wn = fma(a.lam, un, (double)t + (double)c);
-          wv[e] = wn;
-          wu = wn * un;
+          if constexpr (KEEP) pf[e] = fmaf(s_be[r], pf[e], zf[e]);  // as in the product
+          const double pd = (double)pf[e], qn = fma(a.lam, pd, (double)t + (double)c);
+          p[e] = pd;
+          q[e] = qn;
+          pq = qn * pd;
         }
-        wu = col_sum(wu);
-        if (mine && ri == 0) red_add(sums + r * 4 + 2, wu);
+        pq = col_sum(pq);
+        if (mine && ri == 0) red_add(sums + r * 4 + 2, pq);
       }
       if (g + 1 < a.groups) __syncthreads();  // the partial sums are written again
     }
     gb.arrive(0);
+    // off the path to the next sums: the reciprocal that the next beta takes
+    if (warp == 0) {
+      if (on) s_inv[lane] = fabs(rz) > 1e-300 ? 1.0 / rz : 0.0;
+      if (it == 0 && lane < R) s_lim[lane] = a.tol2 * __ldcg(sums + lane * 4 + 1);
+      s_on[lane] = on;
+      c_its += on;
+    }
     if (!gb.leave()) return;
-    // alpha and beta from the sums of all CTAs, one lane a column: an FP64
-    // division costs a warp the same for one lane as for 32
+    // alpha by one lane a column: an FP64 division costs a warp the same for
+    // one lane as for 32
     if (tid < R) {
-      const double ru = __ldcg(sums + tid * 4), rr = __ldcg(sums + tid * 4 + 1), wu = __ldcg(sums + tid * 4 + 2);
-      if (it == 0) c_lim = a.tol2 * rr;
-      c_on = c_on && (it == 0 || rr > c_lim);
-      if (c_on) {
-        const double beta = ru * c_inv, pq = fma(-beta * beta, c_pq, wu);
-        s_al[tid] = pq != 0.0 ? ru / pq : 0.0;
-        s_be[tid] = beta;
-        c_pq = pq;
-        c_ru = ru;
-        c_its += 1;
-      }
-      s_on[tid] = c_on;
+      const double pq = __ldcg(sums + tid * 4 + 2);
+      s_al[tid] = pq != 0.0 ? rz / pq : 0.0;
       // slot it + 2 was last read before the sums just met
       if (blockIdx.x == 0)
         for (int q = 0; q < 3; ++q) __stcg(a.sums + ((size_t)((it + 2) % 3) * R + tid) * 4 + q, 0.0);
     }
     __syncthreads();
-    // x, r, p, s and the next u
+    // x, r and the next z
     for (int cw = warp * (32 / a.gl), r = col0; cw < R; cw += cstep, r += cstep) {
       const bool mine = r < R && ri < nrow;
       if (mine && s_on[r]) {
-        const double beta = s_be[r], al = s_al[r];
+        const double al = s_al[r];
         const int e = r * a.nr + ri;
-        const double pn = fma(beta, p[e], u[e]), sn = fma(beta, s[e], wv[e]);
-        p[e] = pn;
-        s[e] = sn;
-        x[e] = fma(al, pn, x[e]);
-        rv[e] = fma(-al, sn, rv[e]);
+        x[e] = fma(al, p[e], x[e]);
+        rv[e] = fma(-al, q[e], rv[e]);
       }
       publish(r, mine, (it + 1) % 3);
     }
@@ -392,7 +449,7 @@ Shape shape_of(int64_t N, int R, int sm) {
       s.rh = v;
       if (2 * v * s.groups >= R) break;
     }
-    const size_t fixed = ((size_t)6 * s.nr * R + s.nr + 1) * 8 + (size_t)cbs * s.nr * 2 * s.rh * 4;
+    const size_t fixed = ((size_t)4 * s.nr * R + s.nr) * 8 + ((size_t)2 * s.nr * R + (size_t)cbs * s.nr * 2 * s.rh) * 4;
     const size_t room = (size_t)226 * 1024, row = (size_t)s.npad * 4;
     if (fixed > room) continue;
     s.res = (int)std::min<size_t>(s.nr, (room - fixed) / row);
@@ -402,16 +459,16 @@ Shape shape_of(int64_t N, int R, int sm) {
   return s;
 }
 
-template <int RH, int MAXT, bool STREAM>
+template <int RH, int MAXT, bool STREAM, bool KEEP>
 cudaError_t launch(const Args& a, const Shape& s, cudaStream_t st) {
-  auto kern = k_cg_resident<RH, MAXT, STREAM>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
+  auto kern = k_cg_resident<RH, MAXT, STREAM, KEEP>;
+  const cudaError_t e = nk_smem_optin(kern, s.smem);
   if (e != cudaSuccess) return e;
   void* args[] = {const_cast<Args*>(&a)};
   return cudaLaunchCooperativeKernel(kern, dim3((unsigned)s.grid), dim3((unsigned)s.threads), args, s.smem, st);
 }
 
-// The workspace: barrier, status, sums; the published u follows.
+// The workspace: barrier, status, sums; the published vector follows.
 size_t carve(int R, char* w, Args* a) {
   const size_t sums = 256, P = sums + ((size_t)12 * R * 8 + 255) / 256 * 256;
   if (a) {
@@ -454,29 +511,31 @@ cudaError_t nk_cg_resident(const float* K, int64_t ldk, int64_t N, int R, const 
   a.tol2 = tol * tol;
   a.maxit = maxit;
   a.iters = iters;
-  // barrier, sums and the padding of the published u
+  // barrier, sums and the padding of the published vector
   cudaError_t e = cudaMemsetAsync(ws, 0, nk_cg_resident_bytes(N, R, sm), st);
   if (e != cudaSuccess) return e;
   if (s.res < s.nr) {
     switch (s.rh) {
-      case 4: return launch<4, 384, true>(a, s, st);
-      case 5: return launch<5, 384, true>(a, s, st);
-      default: return launch<8, 384, true>(a, s, st);
+      case 4: return launch<4, 384, true, false>(a, s, st);
+      case 5: return launch<5, 384, true, false>(a, s, st);
+      default: return launch<8, 384, true, false>(a, s, st);
     }
   }
   if (s.threads > 512) {
+    if (s.groups > 1) return s.rh == 4 ? launch<4, 768, false, false>(a, s, st) : launch<5, 768, false, false>(a, s, st);
     switch (s.rh) {
-      case 1: return launch<1, 768, false>(a, s, st);
-      case 2: return launch<2, 768, false>(a, s, st);
-      case 4: return launch<4, 768, false>(a, s, st);
-      default: return launch<5, 768, false>(a, s, st);
+      case 1: return launch<1, 768, false, true>(a, s, st);
+      case 2: return launch<2, 768, false, true>(a, s, st);
+      case 4: return launch<4, 768, false, true>(a, s, st);
+      default: return launch<5, 768, false, true>(a, s, st);
     }
   }
+  if (s.groups > 1) return s.rh == 5 ? launch<5, 512, false, false>(a, s, st) : launch<8, 512, false, false>(a, s, st);
   switch (s.rh) {
-    case 1: return launch<1, 512, false>(a, s, st);
-    case 2: return launch<2, 512, false>(a, s, st);
-    case 4: return launch<4, 512, false>(a, s, st);
-    case 5: return launch<5, 512, false>(a, s, st);
-    default: return launch<8, 512, false>(a, s, st);
+    case 1: return launch<1, 512, false, true>(a, s, st);
+    case 2: return launch<2, 512, false, true>(a, s, st);
+    case 4: return launch<4, 512, false, true>(a, s, st);
+    case 5: return launch<5, 512, false, true>(a, s, st);
+    default: return launch<8, 512, false, true>(a, s, st);
   }
 }
