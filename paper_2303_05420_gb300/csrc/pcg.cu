@@ -1011,14 +1011,15 @@ cudaGraphExec_t capture_block(const Pcg& c, double* Xc, int steps, int64_t* per_
 // CG on (K + lam I) Xc = B from Xc = 0 until every column's recursive
 // residual is below tol (relative to ||B||) or maxit iterations; *its = the
 // iterations performed (max over columns).  `graph` replays NK_CHECK_EVERY
-// iterations into Xc (or is null); hflag is pinned host memory.
+// iterations into Xc (or is null); hflag is pinned host memory.  tol_long: the
+// tolerance that a resident run settles for once it gets long.
 template <bool F64>
-cudaError_t cg_run(const Pcg& c, const double* B, double* Xc, double tol, int maxit,
+cudaError_t cg_run(const Pcg& c, const double* B, double* Xc, double tol, double tol_long, int maxit,
                    cudaGraphExec_t graph, int64_t per_block, int* hflag, double* hsc, int* its) {
   if (!F64 && c.res) {
     ++*c.nlaunch;
-    cudaError_t e = nk_cg_resident(c.K, c.ldk, c.N, c.R, B, c.minv, Xc, c.lam, tol, maxit, c.sc + SC_ITER * c.R, c.res,
-                                   c.sm, c.st);
+    cudaError_t e = nk_cg_resident(c.K, c.ldk, c.N, c.R, B, c.minv, Xc, c.lam, tol, tol_long, maxit,
+                                   c.sc + SC_ITER * c.R, c.res, c.sm, c.st);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(hsc, c.sc + SC_ITER * c.R, sizeof(double) * c.R, cudaMemcpyDeviceToHost, c.st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(hflag, (int*)c.res + 1, sizeof(int), cudaMemcpyDeviceToHost, c.st);
@@ -1081,8 +1082,12 @@ cudaError_t cg_run(const Pcg& c, const double* B, double* Xc, double tol, int ma
 // columns, tol 1e-10) the sweeps fell from 7 to 3 and the iterations from 195
 // to 178, 179, 171, and likewise from N = 600 to 2600; 1e-4 ends so close to
 // the rounding that two runs' counts differ by up to 2%, so 1e-3 is taken.
-// Where a sweep falls short of what it was asked for by a factor of four, the
-// rounding has set the level, and the next ones ask for what was reached.
+// A sweep of more than NK_LONG_RUN iterations settles for 3e-2 all the same: in
+// an ill-conditioned system the iterations from there to 1e-3 are the many that
+// the rounding makes worthless (kappa 4e7, 600 points: 13,200 iterations with
+// graph replays, 14,700 with 1e-3 throughout, 12,800 so; kappa 7e6, 1000 points:
+// 3,130, 3,720 and 3,300).  Where a sweep falls short of what it was asked for by
+// a factor of four, the next ones ask for what was reached.
 #define NK_ETA_FLOOR_RESIDENT 1e-3
 
 void nk_pcg_free_host(nk_handle* h) {
@@ -1271,10 +1276,11 @@ nk_status nk_pcg_impl(nk_handle* h, const float* K, int64_t ldk, int64_t N, cons
       if (c.res && outer > 0 && worst > 4.0 * asked * before)
         floor = std::min(std::max(worst / before, floor), NK_ETA_FLOOR);
       const double eta = std::min(std::max(0.5 * tol / worst, floor), 0.5);
+      const double eta_long = std::min(std::max(0.5 * tol / worst, NK_ETA_FLOOR), 0.5);
       asked = eta;
       before = worst;
       int its = 0;
-      e = cg_run<false>(c, c.B2, D, eta, maxit - total_it, graph, per_block, hflag, hsc, &its);
+      e = cg_run<false>(c, c.B2, D, eta, eta_long, maxit - total_it, graph, per_block, hflag, hsc, &its);
       if (e != cudaSuccess) break;
       total_it += its;
       ++h->launches;
@@ -1288,8 +1294,8 @@ nk_status nk_pcg_impl(nk_handle* h, const float* K, int64_t ldk, int64_t N, cons
     const double worst = e == cudaSuccess ? worst_rel() : 0.0;
     if (e == cudaSuccess && worst > tol) {
       const double eta = tol / worst;
-      e = f64 ? cg_run<true>(c, c.B2, D, eta, maxit, graph, per_block, hflag, hsc, &total_it)
-              : cg_run<false>(c, c.B2, D, eta, maxit, graph, per_block, hflag, hsc, &total_it);
+      e = f64 ? cg_run<true>(c, c.B2, D, eta, eta, maxit, graph, per_block, hflag, hsc, &total_it)
+              : cg_run<false>(c, c.B2, D, eta, eta, maxit, graph, per_block, hflag, hsc, &total_it);
       if (e == cudaSuccess) {
         ++h->launches;
         k_add<<<(unsigned)std::min<int64_t>((NR + 255) / 256, 4 * c.sm), 256, 0, st>>>(NR, A, D);
@@ -1300,8 +1306,8 @@ nk_status nk_pcg_impl(nk_handle* h, const float* K, int64_t ldk, int64_t N, cons
     }
     if (e == cudaSuccess) converged = worst_rel() <= tol;
   } else {
-    e = f64 ? cg_run<true>(c, Y, A, tol, maxit, graph, per_block, hflag, hsc, &total_it)
-            : cg_run<false>(c, Y, A, tol, maxit, graph, per_block, hflag, hsc, &total_it);
+    e = f64 ? cg_run<true>(c, Y, A, tol, tol, maxit, graph, per_block, hflag, hsc, &total_it)
+            : cg_run<false>(c, Y, A, tol, tol, maxit, graph, per_block, hflag, hsc, &total_it);
     if (e == cudaSuccess) e = true_residual(c, Y, A, c.B2, f64);
     if (e == cudaSuccess) e = read_sc();
     if (e == cudaSuccess) converged = worst_rel() <= tol;

@@ -62,6 +62,7 @@ struct Args {
   double* sums;         // [3 slots][R][4]: (r, z), (r, r), (p, A p), unused
   unsigned* bar;        // barrier count; bar[1]: status
   double lam, tol2;
+  double tol2_long;     // in place of tol2 from iteration NK_LONG_RUN on
   int maxit;
   double* iters;        // [R] iterations of each column
 };
@@ -141,8 +142,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_resident(const __grid_constant__
   const int pstride = a.nr * 2 * RH;
   // this thread's row and its first column; the columns repeat every cstep
   const int ri = lane & (a.gl - 1), col0 = warp * (32 / a.gl) + lane / a.gl, cstep = (T >> 5) * (32 / a.gl);
-  int c_its = 0;  // iterations of column `lane`, warp 0
-  // per column: alpha, beta, 1 / (r, z), tol^2 (b, b), whether it goes on
+  int c_its = 0;      // column `lane`, warp 0: its iterations
+  double c_bb = 0.0;  // and (b, b)
+  // per column: alpha, 1 / (r, z), tol^2 (b, b), beta, whether it goes on
   __shared__ double s_al[32], s_inv[32], s_lim[32];
   __shared__ float s_be[32];
   __shared__ int s_on[32];
@@ -381,7 +383,11 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_resident(const __grid_constant__
     // off the path to the next sums: the reciprocal that the next beta takes
     if (warp == 0) {
       if (on) s_inv[lane] = fabs(rz) > 1e-300 ? 1.0 / rz : 0.0;
-      if (it == 0 && lane < R) s_lim[lane] = a.tol2 * __ldcg(sums + lane * 4 + 1);
+      if (it == 0 && lane < R) {
+        c_bb = __ldcg(sums + lane * 4 + 1);
+        s_lim[lane] = a.tol2 * c_bb;
+      }
+      if (it == NK_LONG_RUN) s_lim[lane] = a.tol2_long * c_bb;
       s_on[lane] = on;
       c_its += on;
     }
@@ -488,8 +494,8 @@ size_t nk_cg_resident_bytes(int64_t N, int R, int sm) {
 }
 
 cudaError_t nk_cg_resident(const float* K, int64_t ldk, int64_t N, int R, const double* B, const double* minv,
-                           double* X, double lam, double tol, int maxit, double* iters, void* ws, int sm,
-                           cudaStream_t st) {
+                           double* X, double lam, double tol, double tol_long, int maxit, double* iters, void* ws,
+                           int sm, cudaStream_t st) {
   const Shape s = shape_of(N, R, sm);
   if (!s.ok) return cudaErrorNotSupported;
   Args a = {};
@@ -509,6 +515,7 @@ cudaError_t nk_cg_resident(const float* K, int64_t ldk, int64_t N, int R, const 
   carve(R, reinterpret_cast<char*>(ws), &a);
   a.lam = lam;
   a.tol2 = tol * tol;
+  a.tol2_long = tol_long * tol_long;
   a.maxit = maxit;
   a.iters = iters;
   // barrier, sums and the padding of the published vector

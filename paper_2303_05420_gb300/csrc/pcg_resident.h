@@ -9,8 +9,10 @@
 // Workspace of a run; 0 for an N and R that it does not take.
 size_t nk_cg_resident_bytes(int64_t N, int R, int sm);
 // CG on (K + lam I) X = B from X = 0 until every column's recursive residual
-// is at most tol ||B|| or maxit iterations; iters[R] (device) receives the
-// columns' counts, the second unsigned of ws is nonzero if a wait ran out.
+// is at most tol ||B|| (tol_long ||B|| in iterations past NK_LONG_RUN) or maxit
+// iterations; iters[R] (device) receives the columns' counts, the second
+// unsigned of ws is nonzero if a wait ran out.
+#define NK_LONG_RUN 256
 cudaError_t nk_cg_resident(const float* K, int64_t ldk, int64_t N, int R, const double* B, const double* minv,
-                           double* X, double lam, double tol, int maxit, double* iters, void* ws, int sm,
-                           cudaStream_t st);
+                           double* X, double lam, double tol, double tol_long, int maxit, double* iters, void* ws,
+                           int sm, cudaStream_t st);

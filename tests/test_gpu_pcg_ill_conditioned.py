@@ -58,3 +58,19 @@ def test_plain_fp32_solve(n, dim, ell, ridge):
     _, _, rel = h.pcg_solve(K, Y, lam, **kw)
     _, _, graph = h.pcg_solve(K, Y.repeat(1, 11).contiguous(), lam, **kw)
     assert max(rel) <= 3 * max(graph)
+
+
+@pytest.mark.parametrize("n,dim,ell,ridge", [(600, 8, 4.0, 1e-5), (1000, 4, 3.0, 1e-4)])
+def test_long_sweeps_settle_early(n, dim, ell, ridge):
+    """A refinement sweep that gets long stops at the graph-replayed run's level
+    (3e-2), so that the solve takes no more iterations than that run: at most
+    256 in the first sweep, before it shows, and 5 % for the rounding."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2303_05420_gb300.api import Handle
+
+    h = Handle()
+    K, lam, Y = _problem(n, dim, ell, ridge, 3)
+    _, its, _ = h.pcg_solve(K, Y, lam, tol=1e-8, maxit=60000, refine_max=40)
+    _, graph, _ = h.pcg_solve(K, Y.repeat(1, 11).contiguous(), lam, tol=1e-8, maxit=60000, refine_max=40)
+    assert its <= 1.05 * graph + 256
