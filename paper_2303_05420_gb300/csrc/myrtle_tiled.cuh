@@ -205,10 +205,6 @@ struct TiledParams {
   long long wait_limit;           // polls (~0.25-1 us each) before a wait gives up
 };
 
-__device__ __forceinline__ void red_v4(float* a, float x, float y, float z, float w) {
-  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(a), "f"(x), "f"(y), "f"(z), "f"(w)
-               : "memory");
-}
 __device__ __forceinline__ void red_v2(float* a, float x, float y) {
   asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(a), "f"(x), "f"(y) : "memory");
 }

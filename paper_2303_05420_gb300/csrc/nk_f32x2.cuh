@@ -62,24 +62,13 @@ __device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
 // c)^{3/2} B(c) / pi, one multiplication fewer than J, with pi in the tables'
 // folded factor (relative error of J / pi with these FP32 coefficients 4.0e-8;
 // nk_J01_f32's constants give 4.9e-8).
-#ifndef V_CONST
-#define V_CONST 0
-#endif
-#if V_CONST == 1
-__constant__ float2 nk_kB[7] = {{-2.236311266e-04f, -2.236311266e-04f}, {9.384872974e-04f, 9.384872974e-04f}, {-2.355845412e-03f, -2.355845412e-03f}, {5.969292484e-03f, 5.969292484e-03f}, {-2.253424563e-02f, -2.253424563e-02f}, {3.183098733e-01f, 3.183098733e-01f}, {1.f, 1.f}};
-#define KB(i, v) (*reinterpret_cast<const f2*>(&nk_kB[i]))
-#define KONE KB(6, 1.f)
-#else
-#define KB(i, v) f2_dup(v)
-#define KONE f2_dup(1.f)
-#endif
 __device__ __forceinline__ f2 nk_Bpi_poly2(f2 c) {
-  f2 p = KB(0, -2.236311266e-04f);
-  p = f2_fma(p, c, KB(1, 9.384872974e-04f));
-  p = f2_fma(p, c, KB(2, -2.355845412e-03f));
-  p = f2_fma(p, c, KB(3, 5.969292484e-03f));
-  p = f2_fma(p, c, KB(4, -2.253424563e-02f));
-  p = f2_fma(p, c, KB(5, 3.183098733e-01f));
+  f2 p = f2_dup(-2.236311266e-04f);
+  p = f2_fma(p, c, f2_dup(9.384872974e-04f));
+  p = f2_fma(p, c, f2_dup(-2.355845412e-03f));
+  p = f2_fma(p, c, f2_dup(5.969292484e-03f));
+  p = f2_fma(p, c, f2_dup(-2.253424563e-02f));
+  p = f2_fma(p, c, f2_dup(3.183098733e-01f));
   return p;
 }
 
@@ -94,7 +83,7 @@ __device__ __forceinline__ f2 nk_u32(f2 u) {
 // factors 1 / sqrt(q) is infinite, c infinite or (K = 0) a NaN, and such a
 // pixel pair, which adds b b' J ~ 1e-39, would spoil the whole entry.
 __device__ __forceinline__ f2 nk_Jpi01_2(f2 c) {
-  return f2_fma(nk_u32(f2_sub(KONE, c)), nk_Bpi_poly2(c), c);
+  return f2_fma(nk_u32(f2_sub(f2_dup(1.f), c)), nk_Bpi_poly2(c), c);
 }
 
 // J(c) / pi for any c on both halves (nk_J_f32; c beyond [-1, 1] counts as the
@@ -103,7 +92,7 @@ __device__ __forceinline__ f2 nk_Jpi01_2(f2 c) {
 __device__ __forceinline__ f2 nk_Jpi_2(f2 c) {
   const float c0 = f2_lo(c), c1 = f2_hi(c);
   const f2 a = f2_make(fminf(fabsf(c0), 1.f), fminf(fabsf(c1), 1.f));
-  return f2_fma(nk_u32(f2_sub(KONE, a)), nk_Bpi_poly2(a), f2_make(__saturatef(c0), __saturatef(c1)));
+  return f2_fma(nk_u32(f2_sub(f2_dup(1.f), a)), nk_Bpi_poly2(a), f2_make(__saturatef(c0), __saturatef(c1)));
 }
 
 // asin(c) for c in [-1, 1] (nk_asin_f32; values outside by rounding act as
