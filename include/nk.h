@@ -162,7 +162,8 @@ nk_status nk_self_diag(nk_handle* h, const nk_arch* arch, const nk_params* prm,
  * (the CV8 listing: one stage of convs, no pools) MIXED carries only the
  * p = p' diagonal of each pair, which the diagonal stencil keeps closed: H
  * in {8, 16, 32}, W <= 32, ReLU or Erf, C <= 4; one warp per two pairs, FP32
- * recursion, FP64 readout sum.  Other valid requests there return
+ * recursion, the readout sum in two floats a column (FP64 where those leave
+ * FP32), then FP64.  Other valid requests there return
  * NK_ERR_UNSUPPORTED; the layer-wise PLAIN forms take every architecture.  At 64x64
  * MIXED runs the tiled form: stage-0 tasks over row bands and groups of
  * super-plane shifts, the pooled stage-1 tensor of each pair (4 MB) in a

@@ -59,15 +59,23 @@ __device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
 }
 
 // nk_B_poly / pi on both halves: the maps below give J / pi = c + (1 -
-// c)^{3/2} B(c) / pi, one multiplication fewer than J, with pi in the tables'
+// c)^{3/2} B(c) / pi, one multiplication fewer than J, with pi in the layers'
 // folded factor (relative error of J / pi with these FP32 coefficients 4.0e-8;
 // nk_J01_f32's constants give 4.9e-8).
+//
+// DEEP: a fit with next to no mean error (4.3e-8 at c = 0, 1e-8 from c = 0.3 on;
+// csrc/fit_jpos.py pi), for the Flatten readout of many layers without a pool,
+// where errors of one sign add up: 2.4e-8 (rms, eight layers of 32x32, 300 x 250
+// images) against 3.7e-8 with the other one and a rounded layer constant.  The
+// pooled nets are closer with the other one, which their folded factors' rounding
+// offsets (Myrtle-10, 50 x 63: 2.8e-8, and 3.1e-8 with this one).
+template <bool DEEP = false>
 __device__ __forceinline__ f2 nk_Bpi_poly2(f2 c) {
-  f2 p = f2_dup(-2.236311266e-04f);
-  p = f2_fma(p, c, f2_dup(9.384872974e-04f));
-  p = f2_fma(p, c, f2_dup(-2.355845412e-03f));
-  p = f2_fma(p, c, f2_dup(5.969292484e-03f));
-  p = f2_fma(p, c, f2_dup(-2.253424563e-02f));
+  f2 p = f2_dup(DEEP ? -2.113373776e-04f : -2.236311266e-04f);
+  p = f2_fma(p, c, f2_dup(DEEP ? 9.120404720e-04f : 9.384872974e-04f));
+  p = f2_fma(p, c, f2_dup(DEEP ? -2.336561447e-03f : -2.355845412e-03f));
+  p = f2_fma(p, c, f2_dup(DEEP ? 5.963813979e-03f : 5.969292484e-03f));
+  p = f2_fma(p, c, f2_dup(DEEP ? -2.253376879e-02f : -2.253424563e-02f));
   p = f2_fma(p, c, f2_dup(3.183098733e-01f));
   return p;
 }
@@ -82,17 +90,19 @@ __device__ __forceinline__ f2 nk_u32(f2 u) {
 // has no bound there.  Where sqrt(q q') < 2.9e-39 the product a a' of the
 // factors 1 / sqrt(q) is infinite, c infinite or (K = 0) a NaN, and such a
 // pixel pair, which adds b b' J ~ 1e-39, would spoil the whole entry.
+template <bool DEEP = false>
 __device__ __forceinline__ f2 nk_Jpi01_2(f2 c) {
-  return f2_fma(nk_u32(f2_sub(f2_dup(1.f), c)), nk_Bpi_poly2(c), c);
+  return f2_fma(nk_u32(f2_sub(f2_dup(1.f), c)), nk_Bpi_poly2<DEEP>(c), c);
 }
 
 // J(c) / pi for any c on both halves (nk_J_f32; c beyond [-1, 1] counts as the
 // nearer end, a NaN gives 0): J(|c|) + pi min(c, 0) = pi max(c, 0) + (1 -
 // |c|)^{3/2} B(|c|).
+template <bool DEEP = false>
 __device__ __forceinline__ f2 nk_Jpi_2(f2 c) {
   const float c0 = f2_lo(c), c1 = f2_hi(c);
   const f2 a = f2_make(fminf(fabsf(c0), 1.f), fminf(fabsf(c1), 1.f));
-  return f2_fma(nk_u32(f2_sub(f2_dup(1.f), a)), nk_Bpi_poly2(a), f2_make(__saturatef(c0), __saturatef(c1)));
+  return f2_fma(nk_u32(f2_sub(f2_dup(1.f), a)), nk_Bpi_poly2<DEEP>(a), f2_make(__saturatef(c0), __saturatef(c1)));
 }
 
 // asin(c) for c in [-1, 1] (nk_asin_f32; values outside by rounding act as
