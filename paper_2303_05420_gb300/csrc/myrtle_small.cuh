@@ -265,9 +265,7 @@ __global__ void __launch_bounds__(32 * W8, 4) k_myrtle_small8(const __grid_const
         o = entry_layers<2, N2, 32, BIAS>(u, u + 16, t2, P.sb2, lane, sync);
         gap = lane < 16 ? (double)o[lane] : 0.0;
       } else {
-        float s = 0.f;
-        for (int e = lane; e < 256; e += 32) s += o[e];
-        gap = (double)s;
+        for (int e = lane; e < 256; e += 32) gap += (double)o[e];
       }
     }
     gap = warp_total(gap);

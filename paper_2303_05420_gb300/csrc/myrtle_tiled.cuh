@@ -557,18 +557,31 @@ struct Band {
     __syncwarp();
   }
 
-  __device__ __forceinline__ static float row_total(const f2* A) {
+  // Adds a row to a global average: at most four values in FP32 (stage 0 of
+  // 32x32 and 64x64 images, and rows cut into four columns), two elsewhere, then
+  // FP64.  The two halves' sum is split exactly (TwoSum), which beats converting
+  // the halves themselves (160 symmetric 32x32 images 23.2 ms, 23.6 so, 23.1 with
+  // the halves added in FP32) but with a tangent row (NTK of 80 11.75 and 11.69).
+  __device__ __forceinline__ static void add_row(const f2* A, double& sum) {
     f2 s = A[0];
 #pragma unroll
     for (int k = 1; k < COLS; ++k) s = f2_add(s, A[k]);
-    return f2_lo(s) + f2_hi(s);
+    if constexpr (COLS == 1 || (SEED && R >= 32)) {
+      sum += (double)(f2_lo(s) + f2_hi(s));
+    } else if constexpr (NTK) {
+      sum += (double)f2_lo(s) + (double)f2_hi(s);
+    } else {
+      const float a = f2_lo(s), b = f2_hi(s), t = __fadd_rn(a, b), z = __fsub_rn(t, a);
+      sum += (double)t;
+      sum += (double)__fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
+    }
   }
 
   template <int PAR>
   __device__ __forceinline__ void output(const f2 (&A)[COLS], const f2 (&B)[CT], double& gap, double& gapT) {
     if constexpr (GAP) {
-      gap += (double)row_total(A);
-      if constexpr (NTK) gapT += (double)row_total(B);
+      add_row(A, gap);
+      if constexpr (NTK) add_row(B, gapT);
     } else if constexpr (PAR == 0) {
 #pragma unroll
       for (int k = 0; k < COLS; ++k) acc[k] = A[k];
