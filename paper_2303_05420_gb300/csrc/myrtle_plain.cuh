@@ -280,7 +280,7 @@ inline bool conv_layer(const T* in, T* out, int64_t np, int H, int W, int filt, 
     return false;
   }
   auto kern = act ? k_conv_diag<T, true> : k_conv_diag<T, false>;
-  if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  nk_smem_optin(kern, smem);
   const int grp = conv_diag_group(W);
   const int64_t y = std::min<int64_t>((np + grp - 1) / grp, 65535);
   kern<<<dim3((unsigned)(2 * H - 1), (unsigned)y), 256, smem, st>>>(in, out, np, H, W, grp, a, b, addend,
