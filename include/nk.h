@@ -347,13 +347,13 @@ nk_status nk_block_queue(nk_handle* h, const nk_arch* arch, const nk_params* prm
  * MIXED kernel waits for earlier items of its queue (each poll about
  * 0.25-1 us; default 2^22 polls, seconds); the FC kernel's pipeline waits on
  * its mbarriers (each poll a bounded try_wait; default 2^26 polls), and so
- * does the tensor-core first layer of nk_block_backward (FP32, same bound).  A wait
- * that runs out sets NK_ERR_TIMEOUT (read by nk_sync_status), the kernel
+ * does the tensor-core first layer of nk_block_backward (FP32, same bound); the
+ * CTAs of nk_pcg_solve's cooperative CG run wait for each other (each poll about
+ * 0.6 us; default 2^26 polls).  A wait that runs out sets NK_ERR_TIMEOUT (read by
+ * nk_sync_status; returned by nk_pcg_solve itself), the kernel
  * stops taking work, and the results of that call are undefined; the handle
  * stays usable.  The waits a kernel makes before it exits, for its own copies
- * and tensor-core operations in flight, keep a fixed bound, and so do the grid
- * barriers of nk_pcg_solve's cooperative CG run (2^23 polls; that call itself
- * then returns NK_ERR_TIMEOUT).
+ * and tensor-core operations in flight, keep a fixed bound.
  *   polls >= 0: the bound in polls (0: give up at the first unmet check);
  *   polls < 0: the defaults. */
 nk_status nk_set_wait_limit(nk_handle* h, int64_t polls);

@@ -66,10 +66,13 @@ struct nk_handle {
 };
 
 // Default bounds of the device-side waits: polls of the tiled kernel's
-// dependency waits (each about 0.25-1 us) and of the FC kernel's mbarrier
-// waits (each a try_wait of up to a few us).
+// dependency waits (each about 0.25-1 us), of the FC kernel's mbarrier waits
+// (each a try_wait of up to a few us) and of the resident CG run's grid
+// barriers (about 0.6 us: 40 s, because a CTA of that run may have to wait for
+// another stream's kernel to leave its SM, and the others wait for it).
 #define NK_TILED_WAIT_DEFAULT (1ll << 22)
 #define NK_FC_WAIT_DEFAULT (1u << 26)
+#define NK_PCG_WAIT_DEFAULT (1ll << 26)
 
 nk_status nk_fail(nk_handle* h, nk_status s, const char* fmt, ...);
 nk_status nk_cuda_check(nk_handle* h, cudaError_t e, const char* what);

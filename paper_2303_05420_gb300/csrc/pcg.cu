@@ -800,6 +800,8 @@ struct Pcg {
   int pc_rank;
   double *L, *Ginv, *T, *U;
   void* res;         // workspace of the resident run (pcg_resident.cu), or null
+  long long polls;   // bound of its barriers' waits
+  bool* gave_up;     // set when one ran out
 };
 
 
@@ -1019,13 +1021,16 @@ cudaError_t cg_run(const Pcg& c, const double* B, double* Xc, double tol, double
   if (!F64 && c.res) {
     ++*c.nlaunch;
     cudaError_t e = nk_cg_resident(c.K, c.ldk, c.N, c.R, B, c.minv, Xc, c.lam, tol, tol_long, maxit,
-                                   c.sc + SC_ITER * c.R, c.res, c.sm, c.st);
+                                   c.sc + SC_ITER * c.R, c.res, c.sm, c.polls, c.st);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(hsc, c.sc + SC_ITER * c.R, sizeof(double) * c.R, cudaMemcpyDeviceToHost, c.st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(hflag, (int*)c.res + 1, sizeof(int), cudaMemcpyDeviceToHost, c.st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c.st);
     if (e != cudaSuccess) return e;
-    if (*hflag != 0) return cudaErrorLaunchTimeout;
+    if (*hflag != 0) {
+      *c.gave_up = true;
+      return cudaErrorLaunchTimeout;
+    }
     int mx = 0;
     for (int r = 0; r < c.R; ++r) mx = std::max(mx, (int)hsc[r]);
     *its = mx;
@@ -1113,6 +1118,9 @@ nk_status nk_pcg_impl(nk_handle* h, const float* K, int64_t ldk, int64_t N, cons
   c.sm = h->sm_count;
   c.st = st;
   c.nlaunch = &h->launches;
+  bool gave_up = false;
+  c.gave_up = &gave_up;
+  c.polls = h->wait_polls < 0 ? NK_PCG_WAIT_DEFAULT : h->wait_polls;
   const int occ = matvec_prepare(R);
   const int S = choose_splits(N, R, c.sm, occ);
   c.S = S;
@@ -1312,7 +1320,7 @@ nk_status nk_pcg_impl(nk_handle* h, const float* K, int64_t ldk, int64_t N, cons
     if (e == cudaSuccess) e = read_sc();
     if (e == cudaSuccess) converged = worst_rel() <= tol;
   }
-  if (e == cudaErrorLaunchTimeout && c.res) return finish(nk_fail(h, NK_ERR_TIMEOUT, "pcg: a grid barrier gave up"));
+  if (gave_up) return finish(nk_fail(h, NK_ERR_TIMEOUT, "pcg: a grid barrier gave up"));
   if (e != cudaSuccess) return finish(nk_cuda_check(h, e, "pcg"));
   if (iters) *iters = total_it;
   if (!converged) {

@@ -61,6 +61,7 @@ struct Args {
   float* P;             // published z (KEEP) or p, see p_index
   double* sums;         // [3 slots][R][4]: (r, z), (r, r), (p, A p), unused
   unsigned* bar;        // barrier count; bar[1]: status
+  long long polls;      // bound of a barrier's wait
   double lam, tol2;
   double tol2_long;     // in place of tol2 from iteration NK_LONG_RUN on
   int maxit;
@@ -76,14 +77,13 @@ __device__ __forceinline__ int64_t p_index(int npad, int i, int r) {
   return (int64_t)g * npad * 2 * RH + (((i >> 3) * 2 + q / RH) * RH + q % RH) * 8 + (i & 7);
 }
 
-#define NK_WAIT_LIMIT (1ll << 23)
-
 // A barrier of all CTAs, in two halves: arrive() by all threads (everything
 // that they wrote is then on its way), of which the last warp's first thread
 // counts the CTA in and waits, while other warps may go on with work of their
 // own; leave() by all threads, false if the wait ran out.
 struct GridBarrier {
   unsigned* bar;
+  long long polls;  // bound of a wait
   unsigned target;
   bool ok;
   // also: whether `flag` holds in any thread of the CTA
@@ -95,7 +95,7 @@ struct GridBarrier {
       __threadfence();
       atomicAdd(bar, 1u);
       ok = false;
-      for (long long k = 0; k < NK_WAIT_LIMIT && !ok; ++k) {
+      for (long long k = 0; k < polls && !ok; ++k) {
         unsigned v;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
         ok = (int)(v - target) >= 0;
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_cg_resident(const __grid_constant__
   __shared__ double s_al[32], s_inv[32], s_lim[32];
   __shared__ float s_be[32];
   __shared__ int s_on[32];
-  GridBarrier gb = {a.bar, 0, true};
+  GridBarrier gb = {a.bar, a.polls, 0, true};
 
   for (int i = 0; i < res; ++i) {
     const float* src = a.K + (int64_t)(row0 + i) * a.ldk;
@@ -495,7 +495,7 @@ size_t nk_cg_resident_bytes(int64_t N, int R, int sm) {
 
 cudaError_t nk_cg_resident(const float* K, int64_t ldk, int64_t N, int R, const double* B, const double* minv,
                            double* X, double lam, double tol, double tol_long, int maxit, double* iters, void* ws,
-                           int sm, cudaStream_t st) {
+                           int sm, long long polls, cudaStream_t st) {
   const Shape s = shape_of(N, R, sm);
   if (!s.ok) return cudaErrorNotSupported;
   Args a = {};
@@ -513,6 +513,7 @@ cudaError_t nk_cg_resident(const float* K, int64_t ldk, int64_t N, int R, const 
   a.X = X;
   a.gl = s.gl;
   carve(R, reinterpret_cast<char*>(ws), &a);
+  a.polls = polls;
   a.lam = lam;
   a.tol2 = tol * tol;
   a.tol2_long = tol_long * tol_long;
