@@ -380,6 +380,7 @@ struct Band {
   const float* fth;     // folded factor of each layer of this stage (NTK)
   bool dg;              // NTK: the low half is the diagonal super-plane t = (0, 0) of an image with itself
   float b;
+  float ge, geT;        // rounding errors of the rows' sums (add_row)
 
   // the tangent row enters layer j (not the first conv of stage 0)
   template <int j>
@@ -559,29 +560,33 @@ struct Band {
 
   // Adds a row to a global average: at most four values in FP32 (stage 0 of
   // 32x32 and 64x64 images, and rows cut into four columns), two elsewhere, then
-  // FP64.  The two halves' sum is split exactly (TwoSum), which beats converting
-  // the halves themselves (160 symmetric 32x32 images 23.2 ms, 23.6 so, 23.1 with
-  // the halves added in FP32) but with a tangent row (NTK of 80 11.75 and 11.69).
-  __device__ __forceinline__ static void add_row(const f2* A, double& sum) {
+  // FP64.  The two halves' sum is split exactly (TwoSum) and its errors summed in
+  // FP32 until the band's end: an FP64 addition or conversion more a row takes
+  // 1 x 200 images of 32x32 from 438 to 447 us, and the NTK of 80 from 11.62 to
+  // 11.69 ms.  At R = 32 (stage 1 of 64x64) the error's register costs more than
+  // its addition (30 symmetric images 14.89 and 14.66 ms).
+  __device__ __forceinline__ static void add_row(const f2* A, double& sum, float& err) {
     f2 s = A[0];
 #pragma unroll
     for (int k = 1; k < COLS; ++k) s = f2_add(s, A[k]);
     if constexpr (COLS == 1 || (SEED && R >= 32)) {
       sum += (double)(f2_lo(s) + f2_hi(s));
-    } else if constexpr (NTK) {
-      sum += (double)f2_lo(s) + (double)f2_hi(s);
     } else {
       const float a = f2_lo(s), b = f2_hi(s), t = __fadd_rn(a, b), z = __fsub_rn(t, a);
+      const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
       sum += (double)t;
-      sum += (double)__fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
+      if constexpr (R >= 32)
+        sum += (double)e;
+      else
+        err += e;
     }
   }
 
   template <int PAR>
   __device__ __forceinline__ void output(const f2 (&A)[COLS], const f2 (&B)[CT], double& gap, double& gapT) {
     if constexpr (GAP) {
-      add_row(A, gap);
-      if constexpr (NTK) add_row(B, gapT);
+      add_row(A, gap, ge);
+      if constexpr (NTK) add_row(B, gapT, geT);
     } else if constexpr (PAR == 0) {
 #pragma unroll
       for (int k = 0; k < COLS; ++k) acc[k] = A[k];
@@ -663,6 +668,7 @@ struct Band {
   }
 
   __device__ __forceinline__ void run(double& gap, double& gapT) {
+    ge = geT = 0.f;
 #pragma unroll
     for (int j = 0; j < N; ++j)
 #pragma unroll
@@ -724,6 +730,10 @@ struct Band {
       advance((R - N) % STEP);
     }
     if (s1 == R) drain<0>(gap, gapT);
+    if constexpr (GAP && COLS > 1 && R < 32) {
+      gap += (double)ge;
+      if constexpr (NTK) gapT += (double)geT;
+    }
   }
 };
 
