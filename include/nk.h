@@ -406,8 +406,9 @@ nk_status nk_pcg_set_rank(nk_handle* h, int rank);
  *   relres  (host, out, may be NULL) [R] final true relative residuals.
  * With FP32 products, without pivoted Cholesky, R <= 32 and N <= 32 rows per SM
  * (4864 here) a CG run is one cooperative launch that keeps K, or the rows of it
- * that fit, in the SMs' shared memory; other solves replay four to six kernels an
- * iteration from a CUDA graph.
+ * that fit, in the SMs' shared memory; other solves, and these where the device
+ * refuses that launch (a process limited to part of the SMs), replay four to six
+ * kernels an iteration from a CUDA graph.
  * Returns NK_ERR_NOT_CONVERGED (A = best iterate) when maxit is reached.
  * Synchronises `stream`. */
 nk_status nk_pcg_solve(nk_handle* h, const float* K, int64_t ldk, int64_t N,

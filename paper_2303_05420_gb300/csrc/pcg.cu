@@ -1010,32 +1010,36 @@ cudaGraphExec_t capture_block(const Pcg& c, double* Xc, int steps, int64_t* per_
 
 #define NK_CHECK_EVERY 8
 
+// A resident CG run (pcg_resident.cu) into Xc, *its = its iterations (max over
+// columns); tol_long: the tolerance that it settles for once it gets long.
+cudaError_t cg_resident(const Pcg& c, const double* B, double* Xc, double tol, double tol_long, int maxit, int* hflag,
+                        double* hsc, int* its) {
+  cudaError_t e = nk_cg_resident(c.K, c.ldk, c.N, c.R, B, c.minv, Xc, c.lam, tol, tol_long, maxit,
+                                 c.sc + SC_ITER * c.R, c.res, c.sm, c.polls, c.st);
+  if (nk_launch_refused(e)) (void)cudaGetLastError();  // the caller goes on without it
+  if (e != cudaSuccess) return e;
+  ++*c.nlaunch;
+  e = cudaMemcpyAsync(hsc, c.sc + SC_ITER * c.R, sizeof(double) * c.R, cudaMemcpyDeviceToHost, c.st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(hflag, (int*)c.res + 1, sizeof(int), cudaMemcpyDeviceToHost, c.st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c.st);
+  if (e != cudaSuccess) return e;
+  if (*hflag != 0) {
+    *c.gave_up = true;
+    return cudaErrorLaunchTimeout;
+  }
+  int mx = 0;
+  for (int r = 0; r < c.R; ++r) mx = std::max(mx, (int)hsc[r]);
+  *its = mx;
+  return cudaSuccess;
+}
+
 // CG on (K + lam I) Xc = B from Xc = 0 until every column's recursive
 // residual is below tol (relative to ||B||) or maxit iterations; *its = the
 // iterations performed (max over columns).  `graph` replays NK_CHECK_EVERY
-// iterations into Xc (or is null); hflag is pinned host memory.  tol_long: the
-// tolerance that a resident run settles for once it gets long.
+// iterations into Xc (or is null); hflag is pinned host memory.
 template <bool F64>
-cudaError_t cg_run(const Pcg& c, const double* B, double* Xc, double tol, double tol_long, int maxit,
+cudaError_t cg_run(const Pcg& c, const double* B, double* Xc, double tol, int maxit,
                    cudaGraphExec_t graph, int64_t per_block, int* hflag, double* hsc, int* its) {
-  if (!F64 && c.res) {
-    ++*c.nlaunch;
-    cudaError_t e = nk_cg_resident(c.K, c.ldk, c.N, c.R, B, c.minv, Xc, c.lam, tol, tol_long, maxit,
-                                   c.sc + SC_ITER * c.R, c.res, c.sm, c.polls, c.st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(hsc, c.sc + SC_ITER * c.R, sizeof(double) * c.R, cudaMemcpyDeviceToHost, c.st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(hflag, (int*)c.res + 1, sizeof(int), cudaMemcpyDeviceToHost, c.st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c.st);
-    if (e != cudaSuccess) return e;
-    if (*hflag != 0) {
-      *c.gave_up = true;
-      return cudaErrorLaunchTimeout;
-    }
-    int mx = 0;
-    for (int r = 0; r < c.R; ++r) mx = std::max(mx, (int)hsc[r]);
-    *its = mx;
-    return cudaSuccess;
-  }
   *c.nlaunch += 3;
   k_zero<<<1, 256, 0, c.st>>>(c.sc, (int64_t)SC_N * c.R);
   k_set_active<<<1, 256, 0, c.st>>>(c.sc, c.R, tol * tol);
@@ -1250,10 +1254,22 @@ nk_status nk_pcg_impl(nk_handle* h, const float* K, int64_t ldk, int64_t N, cons
   // own earlier A (the captured iteration block writes one fixed array)
   double* Xc = (prec == NK_PREC_MIXED || warm) ? D : A;
   int64_t per_block = 0;
-  if (f64)
-    graph = capture_block<true>(c, Xc, NK_CHECK_EVERY, &per_block);
-  else if (!c.res)
-    graph = capture_block<false>(c, Xc, NK_CHECK_EVERY, &per_block);
+  bool resident = c.res != nullptr, captured = false;
+  // one run from B into Xc; tol_replay: what the sweeps of the replayed form ask for
+  auto run = [&](const double* B, double tol_run, double tol_replay, int limit, int* its) {
+    auto replay = [&](double t) {
+      if (!captured) {
+        captured = true;
+        graph = f64 ? capture_block<true>(c, Xc, NK_CHECK_EVERY, &per_block)
+                    : capture_block<false>(c, Xc, NK_CHECK_EVERY, &per_block);
+      }
+      return f64 ? cg_run<true>(c, B, Xc, t, limit, graph, per_block, hflag, hsc, its)
+                 : cg_run<false>(c, B, Xc, t, limit, graph, per_block, hflag, hsc, its);
+    };
+    return nk_cg_either(
+        &resident, tol_run, tol_replay,
+        [&](double t) { return cg_resident(c, B, Xc, t, tol_replay, limit, hflag, hsc, its); }, replay);
+  };
   bool converged = false;
   int total_it = 0;
   if (prec == NK_PREC_MIXED) {
@@ -1261,7 +1277,7 @@ nk_status nk_pcg_impl(nk_handle* h, const float* K, int64_t ldk, int64_t N, cons
       ++h->launches;
       k_zero<<<(unsigned)std::min<int64_t>((NR + 255) / 256, 4 * c.sm), 256, 0, st>>>(A, NR);
     }
-    double floor = c.res ? NK_ETA_FLOOR_RESIDENT : NK_ETA_FLOOR, asked = 0.0, before = 0.0;
+    double floor = resident ? NK_ETA_FLOOR_RESIDENT : NK_ETA_FLOOR, asked = 0.0, before = 0.0;
     for (int outer = 0;; ++outer) {
       if (outer == 0 && !warm) {
         // A = 0: the residual is Y itself
@@ -1281,14 +1297,16 @@ nk_status nk_pcg_impl(nk_handle* h, const float* K, int64_t ldk, int64_t N, cons
         break;
       }
       if (outer >= refine_max || total_it >= maxit) break;
-      if (c.res && outer > 0 && worst > 4.0 * asked * before)
+      if (!resident)
+        floor = NK_ETA_FLOOR;
+      else if (outer > 0 && worst > 4.0 * asked * before)
         floor = std::min(std::max(worst / before, floor), NK_ETA_FLOOR);
       const double eta = std::min(std::max(0.5 * tol / worst, floor), 0.5);
       const double eta_long = std::min(std::max(0.5 * tol / worst, NK_ETA_FLOOR), 0.5);
       asked = eta;
       before = worst;
       int its = 0;
-      e = cg_run<false>(c, c.B2, D, eta, eta_long, maxit - total_it, graph, per_block, hflag, hsc, &its);
+      e = run(c.B2, eta, eta_long, maxit - total_it, &its);
       if (e != cudaSuccess) break;
       total_it += its;
       ++h->launches;
@@ -1302,8 +1320,7 @@ nk_status nk_pcg_impl(nk_handle* h, const float* K, int64_t ldk, int64_t N, cons
     const double worst = e == cudaSuccess ? worst_rel() : 0.0;
     if (e == cudaSuccess && worst > tol) {
       const double eta = tol / worst;
-      e = f64 ? cg_run<true>(c, c.B2, D, eta, eta, maxit, graph, per_block, hflag, hsc, &total_it)
-              : cg_run<false>(c, c.B2, D, eta, eta, maxit, graph, per_block, hflag, hsc, &total_it);
+      e = run(c.B2, eta, eta, maxit, &total_it);
       if (e == cudaSuccess) {
         ++h->launches;
         k_add<<<(unsigned)std::min<int64_t>((NR + 255) / 256, 4 * c.sm), 256, 0, st>>>(NR, A, D);
@@ -1314,8 +1331,7 @@ nk_status nk_pcg_impl(nk_handle* h, const float* K, int64_t ldk, int64_t N, cons
     }
     if (e == cudaSuccess) converged = worst_rel() <= tol;
   } else {
-    e = f64 ? cg_run<true>(c, Y, A, tol, tol, maxit, graph, per_block, hflag, hsc, &total_it)
-            : cg_run<false>(c, Y, A, tol, tol, maxit, graph, per_block, hflag, hsc, &total_it);
+    e = run(Y, tol, tol, maxit, &total_it);
     if (e == cudaSuccess) e = true_residual(c, Y, A, c.B2, f64);
     if (e == cudaSuccess) e = read_sc();
     if (e == cudaSuccess) converged = worst_rel() <= tol;
