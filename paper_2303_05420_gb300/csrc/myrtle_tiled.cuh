@@ -1219,46 +1219,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_myrtle_tiled(const __grid_cons
   }
 }
 
-// A single block whose items fill a few waves of the grid and a part of one:
-// the pairs of that part get their tasks cut into two or four items (at most
-// one warp task a warp), so that the last wave is as long as its share of the
-// work.  An item's staging, claim and fence, about 0.12 of a whole task's time,
-// are paid by each part: cut only where that is less than what the wave saves.
-// One 32x32 image against 1, 8, 100, 200: 93.5, 104.9, 253, 429 us uncut, 51.0,
-// 55.3, 254, 421 cut.
-inline void split_tail(TiledParams& Q, int64_t* np, int grid, int rounds) {
-  if (Q.n != 1) return;
-  const int nt = Q.nt0[0];
-  const int64_t full = Q.T0 / grid, rest = Q.T0 - full * grid;
-  if (rest == 0 || full >= 24) return;  // a wave in 24 is not worth it
-  const int64_t main = full * grid / nt, tail = Q.G - main;
-  int parts = 1;
-  double best = 0.9;  // the partial wave as it is takes 1
-  for (int n = 2; n <= rounds; n *= 2) {
-    const int64_t waves = (tail * nt * n + grid - 1) / grid;
-    const double cost = (double)waves * (0.88 / n + 0.12) - (double)(tail * nt - rest) / grid;
-    if (cost < best) {
-      best = cost;
-      parts = n;
-    }
-  }
-  if (parts == 1) return;
-  const int b = main > 0 ? 1 : 0;
-  Q.n = b + 1;
-  Q.R[b] = Q.R[0];
-  Q.B[b] = Q.B[0];
-  Q.p0[b] = main;
-  Q.split[b] = parts;
-  Q.wn[b] = Q.wn[0] / parts;
-  Q.nt0[b] = nt * parts;
-  Q.g0[b] = main;
-  Q.f0[b] = main * nt;
-  Q.g0[b + 1] = Q.G;
-  Q.f0[b + 1] = Q.T0 = main * nt + tail * nt * parts;
-  if (b) np[0] = main;
-  np[b] = tail;
-}
-
 template <int N0, int N1, bool BIAS, int NT, int RMAX, int ACT, bool NTK = false, int N2 = 0>
 cudaError_t launch_t(TiledParams& Q, const int64_t* npairs, int sm_count, void* ws, size_t ws_bytes,
                      cudaStream_t st) {
@@ -1283,7 +1243,7 @@ cudaError_t launch_t(TiledParams& Q, const int64_t* npairs, int sm_count, void* 
   constexpr bool TWO = N1 > 0;
   int64_t np[QUEUE_MAX];
   for (int b = 0; b < Q.n; ++b) np[b] = npairs[b];
-  split_tail(Q, np, grid, Q.wn[0] / (NT / 32));
+  if (sched::split_tail(Q, np, grid, Q.wn[0] / (NT / 32))) Q.B[Q.n - 1] = Q.B[0];
   const sched::Plan p = sched::make_plan(TWO, Q.R, np, Q.n, grid, tensors);
   if (p.bytes > ws_bytes) return cudaErrorInvalidValue;
   Q.LAG = p.LAG;
