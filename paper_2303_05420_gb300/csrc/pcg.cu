@@ -862,19 +862,28 @@ int matvec_prepare(int R) {
   return std::max(occ, 1);
 }
 
-// Row splits S of the matvec: one to eight waves of blocks (at least two cost
-// 9.9 ms of 54 at N = 4500, 10 columns, in partial sums), the number of
+// Row splits S of the matvec: up to eight waves of blocks, the number of
 // blocks chosen so that the last wave is nearly full; at least 32 rows per
 // split, and no more splits than keep the FP64 partial sums (S N R words)
 // within a quarter of K's bytes unless that would leave the GPU under one
 // wave (small systems: latency, not bytes, is what counts).
-int choose_splits(int64_t N, int R, int sm, int occ) {
+//
+// At least one wave where the products are FP32: two cost partial sums (80
+// iterations, pivoted Cholesky, N = 4500, 10 columns: 6.8 ms with one, 8.2 with
+// two; 200 columns, N = 1500 12.9 and 14.9, N = 8000 and 100 columns 111 and 119,
+// but N = 4500 and 200 columns 83 and 79).  FP64 products are bound by their pipe
+// and want two waves' even load (N = 3000, 16 columns: 55 and 46 ms; N = 4500, 40
+// columns: 369 and 270), but for one column with a large share of partial sums
+// (N = 4500: 8.4 and 9.3; N = 20000: 133 and 127).
+int choose_splits(int64_t N, int R, int sm, int occ, bool f64) {
   const int64_t colblocks = ((N + 3) / 4 + NK_MV_THREADS - 1) / NK_MV_THREADS;
   const int64_t groups = (R + 15) / 16;
   const int64_t cap = (int64_t)sm * occ;  // resident blocks
   const int64_t per_split = colblocks * groups;
   const int64_t s_rows = std::max<int64_t>(1, std::min<int64_t>(512, N / 32));
-  const int64_t s_lo0 = std::max<int64_t>(1, cap / per_split);
+  const double partial = (double)(2 * cap / per_split) * R * 16.0 / (4.0 * (double)N * (double)groups);
+  const int waves = f64 && (R > 1 || partial < 0.05) ? 2 : 1;
+  const int64_t s_lo0 = std::max<int64_t>(1, waves * cap / per_split);
   const int64_t s_hi0 = std::max<int64_t>(s_lo0, (8 * cap) / per_split);
   const int64_t s_bytes = std::max<int64_t>(1, N / std::max(4 * R, 32));
   const int64_t s_max = std::min<int64_t>(s_rows, std::max<int64_t>(s_bytes, s_lo0));
@@ -882,8 +891,8 @@ int choose_splits(int64_t N, int R, int sm, int occ) {
   int64_t best = s_lo;
   double best_eff = -1.0;
   for (int64_t S = s_lo; S <= s_hi; ++S) {
-    const double waves = (double)(per_split * S) / (double)cap;
-    const double eff = waves / std::ceil(waves);
+    const double w = (double)(per_split * S) / (double)cap;
+    const double eff = w / std::ceil(w);
     if (eff > best_eff + 1e-3) {
       best_eff = eff;
       best = S;
@@ -1126,7 +1135,7 @@ nk_status nk_pcg_impl(nk_handle* h, const float* K, int64_t ldk, int64_t N, cons
   c.gave_up = &gave_up;
   c.polls = h->wait_polls < 0 ? NK_PCG_WAIT_DEFAULT : h->wait_polls;
   const int occ = matvec_prepare(R);
-  const int S = choose_splits(N, R, c.sm, occ);
+  const int S = choose_splits(N, R, c.sm, occ, prec == NK_PREC_PLAIN_FP64);
   c.S = S;
   c.rows_per_split = (int)((N + S - 1) / S);
   const size_t NR = (size_t)N * R;
