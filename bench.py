@@ -74,11 +74,12 @@ def algorithmic_ops_per_entry(hw: int, convs=CONVS, C: int = 3) -> float:
 def executed_ops_per_entry(hw: int, convs=CONVS, C: int = 3) -> float:
     """FP32 lane operations that the packed row stream issues per entry.
 
-    Per pixel pair and layer 16: the stencil is separable (2 FMAs along the
-    row, 2 down the rows), factor products 2, scaling 2, 1 - c 1,
-    (1 - c)^{3/2} 1 beside the square root, the degree-5 polynomial 5, its
-    assembly 1, and 1 for the pair of factors of b b'; seed contraction C,
-    pool or average 1, as above."""
+    Per pixel pair and layer 16 with sigma_b^2 = 0 (one addition more with a
+    bias): the stencil is separable (2 FMAs along the row, 2 down the rows),
+    factor products a a' and b b' 2, scaling by them 2, 1 - c 1, (1 - c)^{3/2} 1
+    beside the square root, the degree-5 polynomial 5, its assembly 1; seed
+    contraction C, pool or average 1, as above.  Clamps, selects and the square
+    root go to other pipes."""
     ops = 0.0
     for s in range(len(convs)):
         if s > 0 and convs[s] == 0:
@@ -584,7 +585,7 @@ def run_ours(args, rank, world, dist):
                      "kernel": "k_myrtle_tiled" if variant == 3 else "k_myrtle_fused",
                      "peak_source": peak_source, "ops_per_entry": ops_entry,
                      # the count is the method's arithmetic (a nine-point stencil, a textbook map), which
-                     # the kernel undercuts, so frac can pass 1; this is the share of the FP32 pipe it uses
+                     # the kernel undercuts, so frac passes 1; this is the share of the FP32 pipe it uses
                      "frac_executed": (achieved_tops / peak_tops * executed_ops_per_entry(hw) / ops_entry
                                        if variant == 3 else None)},
         "e2e": {"value": e2e_val, "unit": "entries/s",
@@ -602,6 +603,7 @@ def run_ours(args, rank, world, dist):
             "pcg_mixed_iters_per_s", "pcg_plain_fp64_iters_per_s", "fc3_gram_ms", "grad_backward_s",
             "queue_graph_ms", "erf_entries_per_s", "cv8_entries_per_s", "config1_entries_per_s", "ntk_mixed_entries_per_s", "ntk10_mixed_entries_per_s"]
     line["summary"] = {"value": value, "e2e": e2e_val, "roofline_frac": achieved_tops / peak_tops,
+                       "roofline_frac_executed": line["roofline"]["frac_executed"],
                        **{k: line.get(k) for k in keys if k in line}}
     if rank == 0:
         print(json.dumps(line), flush=True)
@@ -615,7 +617,8 @@ def pcg_l2_roofline(n: int, iters: float, seconds: float) -> dict:
     peak = load_probe().get("l2_read_GBs")
     return {"bound": "l2", "achieved": gbs, "unit": "GB/s", "peak": peak, "frac": gbs / peak if peak else None,
             "note": "K bytes per iteration / whole-solve time against the probed L2 read bandwidth; the "
-                    "iteration is latency-bound at this size (four dependent launches)"}
+                    "iteration is latency-bound at this size (up to N = 4864 one cooperative launch a CG run, two "
+                    "to three grid barriers an iteration; K is then read once a run)"}
 
 
 def adjoint_layerwise_bytes(convs, hw: int, esize: int = 4, input_sides: int = 2) -> int:
@@ -669,7 +672,7 @@ def adjoint_roofline(seconds: float, pairs_two: int, pairs_one: int, peaks: dict
     return {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
             "bytes_per_pair": per_pair, "traffic": None,
             "note": "layer-fused traffic model (adjoint_layerwise_bytes) x pairs / backward time, against the "
-                    "measured copy bandwidth; the passes are issue-bound, not bandwidth-bound"}
+                    "measured copy bandwidth; the 32x32 passes wait for their loads (issue 50 % forward, 65 % reverse)"}
 
 
 def grad_leg(h, dev, n_sup=100, n_tgt=2048):

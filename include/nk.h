@@ -196,7 +196,8 @@ nk_status nk_block(nk_handle* h, const nk_arch* arch, const nk_params* prm, nk_p
  * products per pair of elements, FP32 accumulation in TMEM, the small
  * cross products first and even / odd K blocks in two accumulators added by
  * the epilogue) with the recursion fused into its epilogue; the per-row
- * self-variances are FP64.
+ * self-variances are sums of exact squares, in two floats a thread and FP64
+ * across threads (FP64 throughout for rows whose squares leave FP32).
  * symmetric: Xa == Xb, equal ranges; tiles below the diagonal are skipped and
  * each entry is stored at (i, j) and (j, i).  depth 0..8.  Uses a handle
  * workspace of (na + nb) * 6 d bytes for the split operands.  A device wait
@@ -394,7 +395,8 @@ nk_status nk_pcg_set_rank(nk_handle* h, int rank);
  *          most 256 products, added in FP64 or in two floats) and FP64
  *          vectors and scalars, A += D (at most refine_max corrections);
  *   prec = NK_PREC_PLAIN_FP32: FP32 K@P, FP64 vectors and scalars, no
- *          refinement;
+ *          refinement (the direction P of a cooperative run, below, is the FP32
+ *          one of its product; iterate and residual are FP64);
  *   prec = NK_PREC_PLAIN_FP64: every product in FP64.
  *   lambda  >= 0: the ridge; < 0: relative ridge, lambda_used =
  *           -lambda * tr(K) / N with tr(K) summed on the device in FP64

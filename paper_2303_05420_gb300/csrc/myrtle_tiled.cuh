@@ -45,8 +45,8 @@
 // 2^22 polls, seconds, by default).
 //
 // What bounds it: instruction issue and the latency of 16 warps an SM, not
-// the FP32 pipe (a 48-image symmetric 32x32 block, 1176 pairs: issue 63 %,
-// FP32 pipe 55 %, shared memory 66 % of their peaks).  The arithmetic is
+// the FP32 pipe (a 48-image symmetric 32x32 block, 1176 pairs: issue 61 %,
+// FP32 pipe 56 %, shared memory 67 % of their peaks).  The arithmetic is
 // packed (f32x2) over two super-planes per lane.  A 160-image symmetric block
 // of 32x32 images: 31.9 ms scalar with one super-plane per lane, 27.6 ms
 // packed, 26.9 ms with maps that give J / pi, 25.6 ms with items decoded in

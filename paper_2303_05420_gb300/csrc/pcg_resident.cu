@@ -20,7 +20,7 @@
 //
 // CG with one reduction (Chronopoulos and Gear: A p and (p, A p) by recurrences)
 // has two crossings everywhere and was faster (12.7 us an iteration at N = 2048,
-// 10 columns, and 13.5 here), but with FP32 products its recurrences drift: at
+// 10 columns, and 13.3 here), but with FP32 products its recurrences drift: at
 // kappa = 7e7 (1000 points, Gaussian kernel) (p, A p) came out negative and
 // the solve diverged where this form converges as the graph-replayed run does.
 // Flags in place of the barriers (a warp waiting for the CTAs that own its
@@ -34,8 +34,11 @@
 // butterfly that folds 16 (row, right-hand side) values at once (15 shuffles,
 // not 80); the warps' sums are added in two floats (TwoSum) and go on in FP64.
 // Short FP32 runs, then wider: as in k_matvec, whose runs are 32 to 256
-// products long.  Vectors, scalars and dot products are FP64; gl lanes (a
-// power of two, at least nr) hold a column's rows, so several columns share a
+// products long.  x, r, A p, scalars and dot products are FP64; the direction is
+// the FP32 one that the product takes (with an FP64 p and its FP32 copy, as in
+// the graph-replayed run, x and r drift apart by the copy's rounding: 600 points,
+// kappa 4e6, products in FP32 alone, residual 1.3e-3 there and 1.1e-3 here).  gl
+// lanes (a power of two, at least nr) hold a column's rows, so several columns share a
 // warp's FP64 instructions, each of which takes its scheduler 64 cycles.
 //
 // Every SM reads the same sums, so all take the same decisions.  Waits are
@@ -429,8 +432,8 @@ struct Shape {
 // All rows in shared memory up to N of about 2,700.  Beyond, up to 32 rows a
 // CTA (a column's lanes; N = 4,864), the rows that fit stay and the others are
 // read in every product, mostly from L2 (K is 81 MB at N = 4500): 34.0 ms with
-// graph replays and 11.8 here at N = 4500, 10 columns, tol 1e-10; at N = 3000,
-// 20 columns 32.5 and 10.3.
+// graph replays and 12.6 here at N = 4500, 10 columns, tol 1e-10; at N = 3000,
+// 20 columns 32.5 and 10.6.
 Shape shape_of(int64_t N, int R, int sm) {
   Shape s = {};
   if (N < 1 || N > (int64_t)32 * sm || N > 8192 || R < 1 || R > 32 || sm < 1) return s;
